@@ -1,0 +1,53 @@
+"""The FP64 step at the ends of the bond law: elastic limits of zero and below
+the normal range, both laws, with the critical stretch from the ratio and from
+the fracture energy, against the oracle.
+
+Tolerance: the damage law's slope is at most k / (s_c - s0) = 25 / 0.025 (nodes
+of 0 and 0.05, ratio 2) on stretches off by at most 10 x 2^-53, so damage agrees
+to 1.2e-12: 2e-12. That error enters the force of each of a node's at most 122
+bonds, none of them more than a fifth of the largest node force: 3e-11."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import pd_workloads as W
+from oracle import core
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(x):
+    return torch.tensor(np.ascontiguousarray(x), device="cuda")
+
+
+@pytest.mark.parametrize("least", [0.0, 3e-310])
+@pytest.mark.parametrize("G_F", [0.0, 5e6])
+@pytest.mark.parametrize("law", [W.LAW_BILINEAR, W.LAW_EXPLINEAR])
+def test_elastic_limit_of_zero(built_lib, law, G_F, least):
+    """Half of the nodes without an elastic limit: bonds between two of them soften under any tension (G_F: the
+    critical stretch is infinite, and the exponential law breaks them)."""
+    pd = built_lib
+    w = W.tiny_beam()
+    g = W.Grid(13, 7, 5, 2.5e-3, 3.01)
+    w = dataclasses.replace(w, grid=g, mat=dataclasses.replace(w.mat, law=law, s_ratio=2.0, G_F=G_F),
+                            bc=dataclasses.replace(w.bc, support_x2=(1, 2 * g.nx - 1), load_x2=g.nx))
+    rng = np.random.default_rng(17)
+    u = rng.normal(0.0, 0.1 * g.dx, (1, g.n_nodes, 3))
+    s0 = np.where(rng.random((1, g.n_nodes)) < 0.5, least, rng.uniform(0.05, 0.15, (1, g.n_nodes)))
+    orow, ocol = core.neighbours(g)
+    row, col = pd.build_neighbours(g)
+    st = pd.State(g, row, col, w.mat, w.bc, batch=1, precision=pd.PREC_FP64)
+    st.reset_f64(_dev(s0))
+    st.load(_dev(u), _dev(np.zeros_like(u)), None, step=0)
+    F, d = st.force().cpu().numpy()[0], st.store()[2].cpu().numpy()[0]
+    st.close()
+    Fo, do, _ = core.Model(w, orow, ocol, s0=s0[0]).force(u[0], np.zeros(len(ocol)))
+    i = np.repeat(np.arange(g.n_nodes), np.diff(orow))
+    both = (s0[0][i] == least) & (s0[0][ocol] == least)
+    assert both.sum() > 100 and ((do > 0) & (do < 1)).any()
+    if law == W.LAW_EXPLINEAR or G_F == 0.0:
+        assert (do[both] == 1.0).sum() > 100
+    assert np.abs(d - do).max() <= 2e-12
+    assert np.abs(F - Fo).max() <= 3e-11 * np.abs(Fo).max()
