@@ -1,6 +1,7 @@
-"""The FP64 step at the ends of the bond law: elastic limits of zero and below
-the normal range, both laws, with the critical stretch from the ratio and from
-the fracture energy, against the oracle.
+"""The FP64 step at the ends of the bond law, against the oracle: elastic limits
+of zero and below the normal range, both laws, with the critical stretch from
+the ratio and from the fracture energy; and bonds compressed to a small part of
+their length.
 
 Tolerance: the damage law's slope is at most k / (s_c - s0) = 25 / 0.025 (nodes
 of 0 and 0.05, ratio 2) on stretches off by at most 10 x 2^-53, so damage agrees
@@ -51,3 +52,31 @@ def test_elastic_limit_of_zero(built_lib, law, G_F, least):
         assert (do[both] == 1.0).sum() > 100
     assert np.abs(d - do).max() <= 2e-12
     assert np.abs(F - Fo).max() <= 3e-11 * np.abs(Fo).max()
+
+
+@pytest.mark.parametrize("shrink", [0.5, 2.0 ** -4, 2.0 ** -10, 2.0 ** -30])
+def test_compressed_bonds(built_lib, shrink):
+    """A body shrunk to `shrink` of its size, its nodes a tenth of the shrunk spacing off. Positions, displacements and
+    their differences are exact (multiples of 2^-56 below 2^-4), so both sides hold the same bond vectors and a bond
+    force is at most 20 roundings off: 20 x 122 x 2^-53 of the largest, below 1e-12."""
+    pd = built_lib
+    w = W.tiny_beam()
+    g = W.Grid(9, 6, 5, 2.0 ** -9, 3.01)
+    w = dataclasses.replace(w, grid=g, bc=dataclasses.replace(w.bc, support_x2=(1, 2 * g.nx - 1), load_x2=g.nx))
+    n = np.arange(g.n_nodes)
+    X = (np.stack([n % g.nx, n // g.nx % g.ny, n // (g.nx * g.ny)], 1) + 0.5) * g.dx
+    noise = np.random.default_rng(3).uniform(-0.1, 0.1, X.shape) * shrink * g.dx
+    u = (shrink - 1.0) * X + np.rint(noise * 2.0 ** 56) * 2.0 ** -56
+    orow, ocol = core.neighbours(g)
+    i = np.repeat(n, np.diff(orow))
+    eta = u[ocol] - u[i]
+    assert np.array_equal(u[i] + eta, u[ocol]) and np.array_equal(X[ocol] - X[i] + eta - eta, X[ocol] - X[i])
+    row, col = pd.build_neighbours(g)
+    st = pd.State(g, row, col, w.mat, w.bc, batch=1, precision=pd.PREC_FP64)
+    st.reset(torch.full((1, g.n_nodes), 1e-4, device="cuda"))
+    st.load(_dev(u[None]), _dev(np.zeros_like(u[None])), None, step=0)
+    F = st.force().cpu().numpy()[0]
+    st.close()
+    Fo, do, _ = core.Model(w, orow, ocol).force(u, np.zeros(len(ocol)))
+    assert not do.any() and np.isfinite(Fo).all()
+    assert np.abs(F - Fo).max() <= 1e-12 * np.abs(Fo).max()
