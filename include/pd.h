@@ -158,7 +158,8 @@ PD_API const char *pd_version(void);
  * row_ptr: device int32[N+1] (always written); col: device int32[cap].
  * n_bonds (host out): number of directed bonds. If col == NULL only row_ptr
  * and n_bonds are produced; if cap < n_bonds, returns PD_ERR_CAP with
- * n_bonds set and col untouched. Host-synchronous (reads back n_bonds).
+ * n_bonds set and col untouched. Host-synchronous: row_ptr and col are complete
+ * on return, whatever stream reads them next.
  * Bit-exact: the list is a pure integer function of the grid. */
 PD_API int pd_build_neighbours(const pd_grid *g, int32_t *row_ptr, int32_t *col, int64_t cap,
                         int64_t *n_bonds, pd_stream stream);

@@ -374,6 +374,7 @@ static int build_rows(const pd_grid *g, int32_t *row_ptr, int32_t *col, int64_t 
     const auto fill = d.all <= 128 ? k_fill_rows<4> : k_fill_rows<0>;
     fill<<<(unsigned)std::min<long long>(need, 8ll * sms), kMeshBlock, 0, s>>>(d, row_ptr, col);
     PD_CHECK_LAUNCH();
+    PD_CHECK_CUDA(cudaStreamSynchronize(s));  // the list is complete on return, for any stream
     return PD_OK;
 }
 
