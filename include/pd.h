@@ -173,7 +173,8 @@ PD_API int pd_build_neighbours(const pd_grid *g, int32_t *row_ptr, int32_t *col,
  * call looks up the array's address on the current device, so no address
  * outlives a cudaDeviceReset. The stream must belong to the current device
  * (PD_ERR_ARG otherwise). Calls that overlap on the GPU share the
- * array and race. Sizes: at most 2^31 - 2 nodes and 2^31 - 1 bonds; larger
+ * array and race for the flag (the count and the rows are each call's own).
+ * Sizes: at most 2^31 - 2 nodes and 2^31 - 1 bonds; larger
  * grids return PD_ERR_ARG (a count-only call detects the bond overflow).
  * Arguments, outputs, synchronisation and errors are those of
  * pd_build_neighbours. */

@@ -343,9 +343,11 @@ extern "C" int pd_last_error(char *buf, size_t len) {
 extern "C" const char *pd_version(void) { return "pd-gb300 0.1 (sm_103a)"; }
 
 // row_ptr, the bond count and, with col, the rows; out2: two words of device
-// scratch.
+// scratch. Where calls in flight together share those (shared), the count, which
+// the rows' space is checked against, comes from the caller's own row_ptr, so
+// that no more than the overflow flag can be lost.
 static int build_rows(const pd_grid *g, int32_t *row_ptr, int32_t *col, int64_t cap, int64_t *n_bonds, int32_t *out2,
-                      cudaStream_t s) {
+                      bool shared, cudaStream_t s) {
     const long long n = (long long)g->nx * g->ny * g->nz;
     const long long nblk = (n + kMeshBlock - 1) / kMeshBlock;
     const GridDev d = make_dev(g);
@@ -359,12 +361,15 @@ static int build_rows(const pd_grid *g, int32_t *row_ptr, int32_t *col, int64_t 
     }
     int32_t h[2] = {0, 0};
     PD_CHECK_CUDA(cudaMemcpyAsync(h, out2, sizeof(h), cudaMemcpyDeviceToHost, s));
+    int32_t total = 0;
+    if (shared) PD_CHECK_CUDA(cudaMemcpyAsync(&total, row_ptr + n, sizeof(total), cudaMemcpyDeviceToHost, s));
     PD_CHECK_CUDA(cudaStreamSynchronize(s));
+    if (!shared) total = h[0];
     PD_REQUIRE(!h[1], "more than 2^31-1 bonds");
-    *n_bonds = h[0];
+    *n_bonds = total;
     if (col == nullptr) return PD_OK;
-    if (cap < h[0]) {
-        set_error("col capacity %lld < %d bonds", (long long)cap, h[0]);
+    if (cap < total) {
+        set_error("col capacity %lld < %d bonds", (long long)cap, total);
         return PD_ERR_CAP;
     }
     int dev = 0, sms = 0;
@@ -385,7 +390,7 @@ extern "C" int pd_build_neighbours(const pd_grid *g, int32_t *row_ptr, int32_t *
     cudaStream_t s = (cudaStream_t)stream;
     Scratch two;
     PD_TRY(scratch_alloc(two, 2 * sizeof(int32_t), s));
-    return build_rows(g, row_ptr, col, cap, n_bonds, (int32_t *)two.p, s);
+    return build_rows(g, row_ptr, col, cap, n_bonds, (int32_t *)two.p, false, s);
 }
 
 extern "C" int pd_bc_codes(const pd_grid *g, const pd_bc *bc, uint8_t *codes, pd_stream stream) {
@@ -402,9 +407,10 @@ extern "C" int pd_bc_codes(const pd_grid *g, const pd_bc *bc, uint8_t *codes, pd
 // Allocation-free variant of pd_build_neighbours.
 //
 // The build needs two words of device scratch beyond its inputs and outputs:
-// the total of the row-pointer scan and its overflow flag.
-// pd_build_neighbours takes them from the scratch pool on every call; this
-// variant keeps them in a file-scope device array instead, for callers that cannot allocate device memory. Its address is
+// the total of the row-pointer scan and its overflow flag. pd_build_neighbours
+// takes them from the scratch pool on every call; this variant keeps them in a
+// file-scope device array instead, for callers that cannot allocate device
+// memory, and reads the total from row_ptr. The array's address is
 // looked up on every call with the current device (cudaGetSymbolAddress), so a
 // context torn down by cudaDeviceReset leaves no stale pointer behind.
 static __device__ __align__(256) int32_t g_noalloc_scratch[64];  // 256 bytes; words 0 and 1: total, overflow
@@ -435,5 +441,5 @@ extern "C" int pd_build_neighbours_noalloc(const pd_grid *g, int32_t *row_ptr, i
     }
     int32_t *two = nullptr;
     PD_TRY(noalloc_scratch(&two));
-    return build_rows(g, row_ptr, col, cap, n_bonds, two, s);  // both words are written on every call
+    return build_rows(g, row_ptr, col, cap, n_bonds, two, true, s);  // both words are written on every call
 }
