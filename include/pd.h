@@ -281,7 +281,8 @@ PD_API int pd_run_to_peak(pd_state *st, int32_t max_steps, double *peak, int32_t
 /* Reverse-mode gradient of J = sum_o dJ_dR[b][o] R^{n0 + obs_steps[o]} of every
  * sample b over a run of n_steps steps from the state's current content
  * (all samples at the same step index n0, as after pd_state_reset or
- * pd_state_load), with respect to the per-node fields s0 and kappa: the exact
+ * pd_state_load; samples that pd_run_to_peak stopped at other steps go on from
+ * their own content at sample 0's step index), with respect to the per-node fields s0 and kappa: the exact
  * discrete adjoint of the step (Eq. PD_EOM_Dynamic, Eq. exp_scalar_force,
  * Eq. exp_damage_parameter, the damped leapfrog update and the reaction), the
  * branch of d_n = max(d_{n-1}, D(s_n)) taken forward kept. The paper has no

@@ -563,9 +563,12 @@ extern "C" int pd_adjoint(pd_state *st, int32_t n_steps, int32_t ckpt_every, int
     const long long N = st->N, nb = st->nb, U3 = (long long)B * N * 3, D1 = (long long)B * nb;
     const int k = std::min(ckpt_every, n_steps);
     const int nseg = (n_steps + k - 1) / k;
-    int32_t n0 = 0;
+    // sample 0's step is the run's; samples that pd_run_to_peak left elsewhere are
+    // taken as they stand
+    std::vector<int32_t> steps(B);
     PD_CHECK_CUDA(cudaStreamSynchronize(s));
-    PD_CHECK_CUDA(cudaMemcpy(&n0, st->step + st->bk_par * B, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    PD_CHECK_CUDA(cudaMemcpy(steps.data(), st->step + st->bk_par * B, B * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    const int32_t n0 = steps[0];
 
     DevBuf<int32_t> obs;
     PD_TRY(dalloc(&obs.p, std::max(n_obs, 1)));
@@ -611,7 +614,7 @@ extern "C" int pd_adjoint(pd_state *st, int32_t n_steps, int32_t ckpt_every, int
         a.iL0q[q] = q ? (float)(1.0 / L0) : 0.f;
     }
     if (st->mat.precision == PD_PREC_MIXED && st->stencil && st->st_sorted)
-        return adjoint_stencil(st, a, n_steps, k, n0, grad_s0, grad_kappa, R_obs, stream);
+        return adjoint_stencil(st, a, n_steps, k, steps.data(), grad_s0, grad_kappa, R_obs, stream);
 
     DevBuf<double> ck_u, ck_v, ck_d, tr_u, tr_d, lu, lun, lv, lF, ld, rbuf;
     // the mixed path's FP32 trajectory: node records (u, s0) per step, damage

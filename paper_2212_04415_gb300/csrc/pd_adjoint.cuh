@@ -68,8 +68,9 @@ int adjoint_gather_obs(int B, int len, int start, int n_obs, const int32_t *obs,
 
 // The adjoint run of a mixed state on the stencil path with ascending CSR
 // rows: forward run with checkpoints every k steps, recomputation and reverse
-// sweep (pd_adjoint's contract; a.obs is on the device).
-int adjoint_stencil(pd_state *st, const AdjArgs &a, int n_steps, int k, int32_t n0, double *grad_s0, double *grad_kappa,
+// sweep (pd_adjoint's contract; a.obs is on the device). steps: [B] the samples'
+// current steps, on the host.
+int adjoint_stencil(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps, double *grad_s0, double *grad_kappa,
                     double *R_obs, pd_stream stream);
 
 }  // namespace pdi

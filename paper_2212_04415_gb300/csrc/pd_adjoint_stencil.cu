@@ -203,6 +203,20 @@ __global__ void __launch_bounds__(256) k_adj_list(const Lay y, int B, const ulon
             if (((r < 64 ? g.x : g.y) >> (r & 63)) & 1ull) words[o++] = (int32_t)word_of<DIM>(y, i, 64 * h + __ffsll(w) - 1);
 }
 
+// The current records of the samples whose step has the other parity than n0
+// (blockIdx.y: sample), into the buffer of n0's.
+__global__ void __launch_bounds__(256) k_adj_align(long long N, long long BN, const int32_t *step, int n0, float4 *rec0,
+                                                   float4 *rec1) {
+    if (!((step[blockIdx.y] ^ n0) & 1)) return;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const size_t t = (size_t)blockIdx.y * N + i;
+    const float4 *from = n0 & 1 ? rec0 : rec1;
+    float4 *to = n0 & 1 ? rec1 : rec0;
+    to[t] = from[t];
+    to[BN + t] = from[BN + t];
+}
+
 // The growing bonds' damage at the current step (blockIdx.y: sample) and, with
 // rec, the node records (u, s0), u = u_hi + u_lo rounded to FP32.
 __global__ void __launch_bounds__(256) k_adj_snap(long long N, long long BN, const long long *base, const int32_t *words,
@@ -541,7 +555,7 @@ struct Bytes {
 
 unsigned blocks_of(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// The state's arrays as one checkpoint. Every live sample is at step n, whose
+// The state's arrays as one checkpoint. Every sample is at step n, whose
 // parity selects the records.
 struct Checkpoint {
     size_t rec, vdf, dmg, dirty;  // bytes
@@ -577,9 +591,10 @@ struct Checkpoint {
 };
 
 template <int DIM>
-int run(pd_state *st, const AdjArgs &a, int n_steps, int k, int32_t n0, double *grad_s0, double *grad_kappa,
+int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps, double *grad_s0, double *grad_kappa,
         double *R_obs, pd_stream stream) {
     cudaStream_t s = (cudaStream_t)stream;
+    const int32_t n0 = steps[0];
     const int B = st->B, nseg = (n_steps + k - 1) / k;
     const long long N = st->N, BN = (long long)B * N;
     PD_REQUIRE(B <= 65535, "at most 65535 samples per state");
@@ -610,6 +625,12 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, int32_t n0, double *
     uint32_t *rows = (uint32_t *)(mem.p + o_rows);
 
     // forward with checkpoints (the step set first clears run bookkeeping, e.g. done flags)
+    if (std::any_of(steps, steps + B, [&](int32_t n) { return (n ^ n0) & 1; })) {
+        k_adj_align<<<dim3(blocks_of(N, 256), B), 256, 0, s>>>(N, BN, st->step + st->bk_par * B, n0, (float4 *)st->rec[0],
+                                                              (float4 *)st->rec[1]);
+        PD_CHECK_LAUNCH();
+        PD_TRY(stencil_refresh_grec(st, s));
+    }
     PD_TRY(state_set_step(st, n0, s));
     for (int g = 0; g < nseg; ++g) {
         const int start = g * k, len = std::min(k, n_steps - start);
@@ -748,10 +769,10 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, int32_t n0, double *
 
 }  // namespace
 
-int adjoint_stencil(pd_state *st, const AdjArgs &a, int n_steps, int k, int32_t n0, double *grad_s0, double *grad_kappa,
-                    double *R_obs, pd_stream stream) {
-    return st->st_dim == 3 ? run<3>(st, a, n_steps, k, n0, grad_s0, grad_kappa, R_obs, stream)
-                           : run<2>(st, a, n_steps, k, n0, grad_s0, grad_kappa, R_obs, stream);
+int adjoint_stencil(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps, double *grad_s0,
+                    double *grad_kappa, double *R_obs, pd_stream stream) {
+    return st->st_dim == 3 ? run<3>(st, a, n_steps, k, steps, grad_s0, grad_kappa, R_obs, stream)
+                           : run<2>(st, a, n_steps, k, steps, grad_s0, grad_kappa, R_obs, stream);
 }
 
 }  // namespace pdi
