@@ -294,8 +294,8 @@ PD_API int pd_run_to_peak(pd_state *st, int32_t max_steps, double *peak, int32_t
  *   grad_s0, grad_kappa: device double[B][N] out (grad_kappa may be NULL)
  *   R_obs:     device double[B][n_obs] out, the forward reactions, or NULL
  * Checkpoints (u, v, d) every ckpt_every steps (k) and recomputes each
- * segment. Device memory, allocated per call (PD_ERR_OOM when unavailable),
- * per sample: for mixed-path states on the stencil path (n_steps / k + 2)
+ * segment. Device memory, allocated per call (PD_ERR_OOM when unavailable, with
+ * the state as it was), per sample: for mixed-path states on the stencil path (n_steps / k + 2)
  * copies of the state's arrays (64 N + 520 N bytes with whole bricks), 16 k N
  * bytes of FP32 node records, 128 N bytes of adjoint state and masks, and per
  * bond whose damage grows in the run (only those carry a damage adjoint)

@@ -590,6 +590,37 @@ struct Checkpoint {
     }
 };
 
+// The run bookkeeping of a state, to put back when a call fails after it has
+// stepped the state.
+struct Bookkeeping {
+    int32_t bk_par, rec_off;
+    static constexpr int kParts = 9;
+    struct Part {
+        void *p;
+        size_t bytes;
+    } part[kParts];
+    explicit Bookkeeping(const pd_state *st) : bk_par(st->bk_par), rec_off(st->rec_off) {
+        const size_t B = st->B;
+        const Part of[kParts] = {{st->step, 8 * B},   {st->done, 8 * B},   {st->pend, 8 * B},
+                                 {st->pk2, 16 * B},   {st->ps2, 8 * B},    {st->status, 4 * B},
+                                 {st->peak, 8 * B},   {st->peak_step, 4 * B}, {st->ticket, 4 * B}};
+        std::copy(of, of + kParts, part);
+    }
+    static size_t bytes(int B) { return (size_t)kParts * 16 * B; }
+    int copy(char *saved, bool back, cudaStream_t s) const {
+        for (const Part &q : part) {
+            PD_CHECK_CUDA(cudaMemcpyAsync(back ? q.p : saved, back ? saved : q.p, q.bytes, cudaMemcpyDeviceToDevice, s));
+            saved += q.bytes;
+        }
+        return PD_OK;
+    }
+    int restore(pd_state *st, char *saved, cudaStream_t s) const {
+        st->bk_par = bk_par;
+        st->rec_off = rec_off;
+        return copy(saved, true, s);
+    }
+};
+
 template <int DIM>
 int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps, double *grad_s0, double *grad_kappa,
         double *R_obs, pd_stream stream) {
@@ -602,7 +633,7 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     const AdjTile T = pick_tile(st->g, Sten<DIM>::kHaloZ);
     const unsigned tiles = (unsigned)(T.ntx * T.nty * T.ntz), threads = 8u * T.ty * T.tz;
     // one allocation: checkpoints and the final state, FP32 node records of a
-    // segment, (lamF, kappa) of two steps, lamu, lamv, reactions, masks and list starts
+    // segment, (lamF, kappa) of two steps, lamu, lamv, reactions, masks, list starts and the run bookkeeping
     size_t off = 0;
     const auto part = [&](size_t bytes) {
         const size_t at = off;
@@ -614,7 +645,8 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
                  o_lv = part(3 * BN * sizeof(double)), o_r = part((size_t)B * k * sizeof(double)),
                  o_rows = part((size_t)tiles * (threads / 32) * kRowWords<DIM> * 32 * sizeof(uint32_t)),
                  o_pm = part(N * sizeof(ulonglong2)), o_gm = part(BN * sizeof(ulonglong2)),
-                 o_km = part(BN * sizeof(ulonglong2)), o_base = part((BN + 1) * sizeof(long long));
+                 o_km = part(BN * sizeof(ulonglong2)), o_base = part((BN + 1) * sizeof(long long)),
+                 o_bk = part(Bookkeeping::bytes(B));
     Bytes mem;
     PD_TRY(dalloc(&mem.p, off));
     const auto ck_at = [&](int g) { return mem.p + o_ck + (size_t)g * ck.bytes(); };
@@ -623,6 +655,9 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     ulonglong2 *pm = (ulonglong2 *)(mem.p + o_pm), *gm = (ulonglong2 *)(mem.p + o_gm), *km = (ulonglong2 *)(mem.p + o_km);
     long long *base = (long long *)(mem.p + o_base);
     uint32_t *rows = (uint32_t *)(mem.p + o_rows);
+
+    const Bookkeeping bk(st);
+    PD_TRY(bk.copy(mem.p + o_bk, false, s));
 
     // forward with checkpoints (the step set first clears run bookkeeping, e.g. done flags)
     if (std::any_of(steps, steps + B, [&](int32_t n) { return (n ^ n0) & 1; })) {
@@ -675,7 +710,13 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     const size_t o_tr = part((size_t)(k + 1) * ng * sizeof(float)), o_ld = part(ng * sizeof(float2)),
                  o_words = part(ng * sizeof(int32_t));
     Bytes gmem;
-    PD_TRY(dalloc(&gmem.p, off));
+    const int grc = dalloc(&gmem.p, off);
+    if (grc != PD_OK) {  // the state as the call found it
+        PD_TRY(ck.restore(st, n0, ck_at(0), s));
+        PD_TRY(bk.restore(st, mem.p + o_bk, s));
+        PD_CHECK_CUDA(cudaStreamSynchronize(s));
+        return grc;
+    }
     float *tr_d = (float *)(gmem.p + o_tr);
     float2 *ld = (float2 *)(gmem.p + o_ld);
     int32_t *words = (int32_t *)(gmem.p + o_words);
