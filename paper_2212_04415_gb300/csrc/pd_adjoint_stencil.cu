@@ -186,10 +186,12 @@ __device__ __forceinline__ long long word_of(const Lay &y, int i, int e) {
     return (((brick * y.wpb + (row >> 1)) * (R / 4) + m / 4) * 32 + (16 * t + 8 * (row & 1) + ix % kSlice)) * 4 + m % 4;
 }
 
-// Damage words of the growing bonds, node after node in row order.
-template <int DIM>
+// Damage words of the growing bonds, node after node in row order. W: 32 bits
+// where a sample's words fit them, 64 above (from 2^25 node places of whole
+// bricks on; every step reads the list).
+template <int DIM, class W>
 __global__ void __launch_bounds__(256) k_adj_list(const Lay y, int B, const ulonglong2 *present, const ulonglong2 *grow,
-                                                  const long long *base, int32_t *words) {
+                                                  const long long *base, W *words) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= y.N * B) return;
     const ulonglong2 g = grow[t];
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(256) k_adj_list(const Lay y, int B, const ulon
     int r = 0;  // row position
     for (int h = 0; h < 2; ++h)
         for (unsigned long long w = h ? P.y : P.x; w; w &= w - 1, ++r)
-            if (((r < 64 ? g.x : g.y) >> (r & 63)) & 1ull) words[o++] = (int32_t)word_of<DIM>(y, i, 64 * h + __ffsll(w) - 1);
+            if (((r < 64 ? g.x : g.y) >> (r & 63)) & 1ull) words[o++] = (W)word_of<DIM>(y, i, 64 * h + __ffsll(w) - 1);
 }
 
 // The current records of the samples whose step has the other parity than n0
@@ -219,7 +221,8 @@ __global__ void __launch_bounds__(256) k_adj_align(long long N, long long BN, co
 
 // The growing bonds' damage at the current step (blockIdx.y: sample) and, with
 // rec, the node records (u, s0), u = u_hi + u_lo rounded to FP32.
-__global__ void __launch_bounds__(256) k_adj_snap(long long N, long long BN, const long long *base, const int32_t *words,
+template <class W>
+__global__ void __launch_bounds__(256) k_adj_snap(long long N, long long BN, const long long *base, const W *words,
                                                   const float *dmg, long long st_len, float *out, const float4 *rec,
                                                   float4 *u4) {
     const int b = blockIdx.y;
@@ -706,9 +709,10 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     PD_CHECK_CUDA(cudaMemcpyAsync(&n_grow, base + BN, sizeof(n_grow), cudaMemcpyDeviceToHost, s));
     PD_CHECK_CUDA(cudaStreamSynchronize(s));
     const size_t ng = (size_t)std::max(n_grow, 1ll);
+    const bool wide = st->st_len > (1ll << 32);  // a sample's damage words
     off = 0;
     const size_t o_tr = part((size_t)(k + 1) * ng * sizeof(float)), o_ld = part(ng * sizeof(float2)),
-                 o_words = part(ng * sizeof(int32_t));
+                 o_words = part(ng * (wide ? sizeof(uint64_t) : sizeof(uint32_t)));
     Bytes gmem;
     const int grc = dalloc(&gmem.p, off);
     if (grc != PD_OK) {  // the state as the call found it
@@ -719,8 +723,12 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     }
     float *tr_d = (float *)(gmem.p + o_tr);
     float2 *ld = (float2 *)(gmem.p + o_ld);
-    int32_t *words = (int32_t *)(gmem.p + o_words);
-    k_adj_list<DIM><<<blocks_of(BN, 256), 256, 0, s>>>(y, B, pm, gm, base, words);
+    uint32_t *words = (uint32_t *)(gmem.p + o_words);
+    uint64_t *words64 = (uint64_t *)(gmem.p + o_words);
+    if (wide)
+        k_adj_list<DIM><<<blocks_of(BN, 256), 256, 0, s>>>(y, B, pm, gm, base, words64);
+    else
+        k_adj_list<DIM><<<blocks_of(BN, 256), 256, 0, s>>>(y, B, pm, gm, base, words);
     PD_CHECK_LAUNCH();
     PD_CHECK_CUDA(cudaMemsetAsync(ld, 0, ng * sizeof(float2), s));
     PD_CHECK_CUDA(cudaMemsetAsync(lu, 0, 3 * BN * sizeof(double), s));
@@ -771,7 +779,10 @@ int run(pd_state *st, const AdjArgs &a, int n_steps, int k, const int32_t *steps
     PD_CHECK_CUDA(cudaFuncSetAttribute(k_adj_bonds_st<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * sizeof(float4) * kMaxCells)));
     const dim3 snap_grid((unsigned)std::max(1, std::min(64, (int)blocks_of(N, 256))), (unsigned)B);
     const auto snap = [&](const float4 *rec, float4 *dst, float *d) -> int {
-        k_adj_snap<<<snap_grid, 256, 0, s>>>(N, BN, base, words, (const float *)st->dmg, st->st_len, d, rec, dst);
+        if (wide)
+            k_adj_snap<<<snap_grid, 256, 0, s>>>(N, BN, base, words64, (const float *)st->dmg, st->st_len, d, rec, dst);
+        else
+            k_adj_snap<<<snap_grid, 256, 0, s>>>(N, BN, base, words, (const float *)st->dmg, st->st_len, d, rec, dst);
         PD_CHECK_LAUNCH();
         return PD_OK;
     };
