@@ -230,7 +230,7 @@ __global__ void k_sell_fill(long long N, const int32_t *row_ptr, const int32_t *
 
 // Damage of every sample in sliced-ELL order from the CSR-order slot table
 // of the stencil damage array (padding slots read slot 0 and are unused).
-__global__ void k_sell_slots(long long len, const int32_t *q_of, const int32_t *slot, int32_t *dslot) {
+__global__ void k_sell_slots(long long len, const int32_t *q_of, const long long *slot, long long *dslot) {
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= len) return;
     const int q = q_of[x];
@@ -246,7 +246,7 @@ constexpr uint8_t kDmgZero = 0, kDmgGrows = 1, kDmgConst = 2;
 // partly used sector per slot from L2. Only slots whose damage grows in the
 // run are gathered (code[] per sample and slot); the bond adjoint reads no
 // other slot of the trajectory.
-__global__ void k_gather_dmg(long long len, long long dlen, const long long *off, const int32_t *dslot,
+__global__ void k_gather_dmg(long long len, long long dlen, const long long *off, const long long *dslot,
                              const uint8_t *code, const float *dmg, float *out) {
     const long long a0 = off[blockIdx.x], a1 = off[blockIdx.x + 1];
     const int b = blockIdx.y;
@@ -624,8 +624,8 @@ extern "C" int pd_adjoint(pd_state *st, int32_t n_steps, int32_t ckpt_every, int
     DevBuf<float4> tr_u4, lF4;
     DevBuf<float> tr_d32;
     DevBuf<float2> ld2;
-    DevBuf<int32_t> slot, q_of, k_of, dslot;
-    DevBuf<long long> sl_off;
+    DevBuf<int32_t> q_of, k_of;
+    DevBuf<long long> sl_off, slot, dslot;
     DevBuf<uint8_t> grow8;  // mixed path: per sample and slot, the damage history code (k_grows)
     long long nsl = 0;  // slices of 32 nodes (mixed path)
     long long SL = 0;  // sliced-ELL slots per sample

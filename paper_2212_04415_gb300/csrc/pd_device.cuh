@@ -460,7 +460,7 @@ int stencil_reset_damage(pd_state *st, cudaStream_t s);
 int stencil_map_damage(const pd_state *st, double *csr, bool to_state, cudaStream_t s);
 // slot of every CSR bond in one sample's stencil damage array (the adjoint
 // gathers its FP32 damage trajectory through it)
-int stencil_slot_table(const pd_state *st, int32_t *slot, cudaStream_t s);
+int stencil_slot_table(const pd_state *st, long long *slot, cudaStream_t s);
 void stencil_fill_args(const pd_state *st, StepArgs &a);
 // the stencil kernel's gather records (u / dx, s0 / 2), both parities, from the state's records
 int stencil_refresh_grec(pd_state *st, cudaStream_t s);

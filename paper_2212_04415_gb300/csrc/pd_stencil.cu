@@ -273,12 +273,12 @@ __global__ void k_stencil_map_any(const int32_t *row_ptr, const int32_t *col, co
 // is a stencil offset: checked when the template is built).
 __global__ void k_stencil_slots(const int32_t *row_ptr, const int32_t *col, const int32_t *coord, long long N,
                                 int nx, int ny, int BY, int BZ, int nbx, int nby, int wpb, int rounds,
-                                const int16_t *box, int32_t *slot) {
+                                const int16_t *box, long long *slot) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     for (int p = row_ptr[i]; p < row_ptr[i + 1]; ++p) {
         const int code = code_of(coord, (int)i, col[p], box);
-        slot[p] = code < 0 ? 0 : (int32_t)slot_of((int)i, code, nx, ny, BY, BZ, nbx, nby, wpb, rounds);
+        slot[p] = code < 0 ? 0 : slot_of((int)i, code, nx, ny, BY, BZ, nbx, nby, wpb, rounds);
     }
 }
 
@@ -545,7 +545,7 @@ int stencil_map_damage(const pd_state *st, double *csr, bool to_state, cudaStrea
     return PD_OK;
 }
 
-int stencil_slot_table(const pd_state *st, int32_t *slot, cudaStream_t s) {
+int stencil_slot_table(const pd_state *st, long long *slot, cudaStream_t s) {
     k_stencil_slots<<<blocks_of(st->N), 256, 0, s>>>(st->row_ptr, st->col_csr, st->coord, st->N, st->g.nx, st->g.ny,
                                                      st->by, st->bz, st->nbx, st->nby, st->st_wpb,
                                                      st->st_dim == 3 ? Sten<3>::kRounds : Sten<2>::kRounds,

@@ -16,11 +16,14 @@ pytestmark = pytest.mark.gpu
 TOP = 30  # rows compared (6 steps reach 18 rows from the load line)
 
 
-def _gradients(pd, nx, ny):
+def _gradients(pd, nx, ny, descending=False):
     w = W.tiny_beam(nx, ny, 2, notch=False)
     w = dataclasses.replace(w, mat=dataclasses.replace(w.mat, s_ratio=1e4))
     g = w.grid
     row, col = pd.build_neighbours(g)
+    if descending:
+        r = row.long()
+        col = col[torch.repeat_interleave(r[:-1] + r[1:] - 1, r.diff()) - torch.arange(col.numel(), device="cuda")]
     st = pd.State(g, row, col, w.mat, w.bc, batch=1, schedule=(2, 16, 1))
     del row, col
     s0 = torch.full((1, g.n_nodes), 1e-7, device="cuda")
