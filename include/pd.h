@@ -360,7 +360,8 @@ PD_API int pd_field_info(const pd_field *f, int32_t *n_modes, double *lambda);
  * with ds0/dg = sigma s0 (lognormal) or the Weibull copula's derivative;
  * g is recomputed in FP64 from xi. xi: device double[B][K]; dJ_ds0: device
  * double[B][N_level]; dJ_dxi: device double[B][K] out (FP64, fixed-order
- * sums). Host-synchronous. */
+ * sums). Device scratch of at most 64 MB whatever the sizes (PD_ERR_OOM when
+ * unavailable). Host-synchronous. */
 PD_API int pd_field_adjoint(const pd_field *f, int32_t level, const double *xi, int32_t B,
                             const double *dJ_ds0, double *dJ_dxi, pd_stream stream);
 

@@ -429,9 +429,15 @@ int adjoint_gather_obs(int B, int len, int start, int n_obs, const int32_t *obs,
 constexpr int kFgMaxK = 256;
 constexpr int kFgThreads = 256;
 constexpr int kFgSamples = 16;  // samples per block
-constexpr int kFgTile = 8192;   // psi values of a block's nodes (64 KB as FP64)
+constexpr int kFgTile = 8192;   // psi values of a tile of nodes (64 KB as FP64)
+// The partial sums are scratch: at most kFgChunks per sample and mode (a block
+// takes several tiles of a grid that has more), for as many samples at a time as
+// kFgScratch holds (16 at least; 1,024 x 256 modes x 16 samples take 32 MB), so
+// large grids and batches need no more memory than small ones.
+constexpr int kFgChunks = 1024;
+constexpr size_t kFgScratch = 64u << 20;
 
-// Nodes per block: a power of two of at most 128 whose psi rows fit the tile.
+// Nodes per tile: a power of two of at most 128 whose psi rows fit the tile.
 static int fg_nodes(int K) {
     int n = 128;
     while (n * K > kFgTile) n /= 2;
@@ -464,61 +470,69 @@ __device__ __forceinline__ void dots_of(int c, int n, const double *p, int ps, c
         dots<1>(n, p, ps, q, qs, a);
 }
 
-// partial[b][chunk][k] = sum over the chunk's nodes of dJ/dg_i Psi_ik (FP64,
-// fixed order), for up to kFgSamples samples of a block. Both contractions
+// partial[b][chunk][k] = sum over the chunk's nodes (`per` tiles of NT, one after
+// the other) of dJ/dg_i Psi_ik (FP64, fixed order), for up to kFgSamples samples
+// of a block. Both contractions
 // (g = Psi xi, then Psi^T dJ/dg) take their operands as FP64 from shared
 // memory, four samples to a register tile, so the FP64 pipe of this part (2
 // lanes an SM) does the products and one conversion per basis value and block;
 // it bounds the kernel: 28,000 nodes x 64 modes x 32 samples are 115M
 // multiply-adds, 0.2 ms. (With the basis read at stride K and converted for
 // every sample, and a block reduction per mode, the call took 0.65 ms.)
-__global__ void __launch_bounds__(kFgThreads) k_field_grad_partial(long long N, int K, int B, int NT, const float *psi,
+__global__ void __launch_bounds__(kFgThreads) k_field_grad_partial(long long N, int K, int B, int NT, int per, const float *psi,
                                                                    const double *xi, const double *dJ_ds0, int marginal,
                                                                    double mu, double sig, double wscale, double m_w,
                                                                    int nchunks, double *partial) {
     extern __shared__ double s_fg[];
     const int b0 = blockIdx.y * kFgSamples, bt = min(kFgSamples, B - b0), chunk = blockIdx.x;
-    const long long i0 = (long long)chunk * NT;
-    const int nt = (int)min((long long)NT, N - i0);
     double *s_psi = s_fg;                              // [node][K + 1]
     double *s_xi = s_psi + (size_t)NT * (K + 1);       // [sample][K]
     double *s_w = s_xi + (size_t)kFgSamples * K;       // [sample][NT]
     const int PS = K | 1;  // odd: a warp of nodes reads without bank conflicts
-    for (int q = threadIdx.x; q < nt * K; q += kFgThreads) s_psi[q / K * PS + q % K] = (double)psi[i0 * K + q];
     for (int q = threadIdx.x; q < bt * K; q += kFgThreads) s_xi[q] = xi[(size_t)b0 * K + q];
-    __syncthreads();
-    // dJ/dg of (node, four samples) per thread; a warp's nodes share their samples
-    const int node = threadIdx.x & (NT - 1);
-    if (node < nt) {
-        for (int s0 = threadIdx.x / NT * 4; s0 < bt; s0 += kFgThreads / NT * 4) {
-            double g[4];
-            const int c = min(4, bt - s0);
-            dots_of(c, K, s_psi + node * PS, 1, s_xi + s0 * K, K, g);
+    for (int tile = 0; tile < per; ++tile) {
+        const long long i0 = ((long long)chunk * per + tile) * NT;
+        if (i0 >= N) break;  // block-uniform
+        const int nt = (int)min((long long)NT, N - i0);
+        if (tile) __syncthreads();  // the tile before has been read
+        for (int q = threadIdx.x; q < nt * K; q += kFgThreads) s_psi[q / K * PS + q % K] = (double)psi[i0 * K + q];
+        __syncthreads();
+        // dJ/dg of (node, four samples) per thread; a warp's nodes share their samples
+        const int node = threadIdx.x & (NT - 1);
+        if (node < nt) {
+            for (int s0 = threadIdx.x / NT * 4; s0 < bt; s0 += kFgThreads / NT * 4) {
+                double g[4];
+                const int c = min(4, bt - s0);
+                dots_of(c, K, s_psi + node * PS, 1, s_xi + s0 * K, K, g);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (j >= c) break;
-                const double dj = dJ_ds0[(size_t)(b0 + s0 + j) * N + i0 + node];
-                double wg;
-                if (marginal == PD_MARG_LOGNORMAL) {
-                    wg = dj * sig * exp(mu + sig * g[j]);
-                } else {
-                    const double q = 0.5 * erfc(g[j] / 1.4142135623730951);
-                    const double pdf = exp(-0.5 * g[j] * g[j]) / 2.5066282746310002;
-                    wg = dj * (wscale / m_w) * pow(-log(q), 1.0 / m_w - 1.0) * pdf / q;
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= c) break;
+                    const double dj = dJ_ds0[(size_t)(b0 + s0 + j) * N + i0 + node];
+                    double wg;
+                    if (marginal == PD_MARG_LOGNORMAL) {
+                        wg = dj * sig * exp(mu + sig * g[j]);
+                    } else {
+                        const double q = 0.5 * erfc(g[j] / 1.4142135623730951);
+                        const double pdf = exp(-0.5 * g[j] * g[j]) / 2.5066282746310002;
+                        wg = dj * (wscale / m_w) * pow(-log(q), 1.0 / m_w - 1.0) * pdf / q;
+                    }
+                    s_w[(s0 + j) * NT + node] = wg;
                 }
-                s_w[(s0 + j) * NT + node] = wg;
             }
         }
-    }
-    __syncthreads();
-    const int nsb = (bt + 3) / 4;
-    for (int q = threadIdx.x; q < K * nsb; q += kFgThreads) {
-        const int k = q % K, s0 = q / K * 4, c = min(4, bt - s0);
-        double v[4];
-        dots_of(c, nt, s_psi + k, PS, s_w + s0 * NT, NT, v);
+        __syncthreads();
+        const int nsb = (bt + 3) / 4;
+        for (int q = threadIdx.x; q < K * nsb; q += kFgThreads) {
+            const int k = q % K, s0 = q / K * 4, c = min(4, bt - s0);
+            double v[4];
+            dots_of(c, nt, s_psi + k, PS, s_w + s0 * NT, NT, v);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (j < c) partial[((size_t)(b0 + s0 + j) * nchunks + chunk) * K + k] = v[j];
+            for (int j = 0; j < 4; ++j)
+                if (j < c) {
+                    double *p = partial + ((size_t)(b0 + s0 + j) * nchunks + chunk) * K + k;
+                    *p = tile ? *p + v[j] : v[j];
+                }
+        }
     }
 }
 
@@ -792,17 +806,24 @@ extern "C" int pd_field_adjoint(const pd_field *f, int32_t level, const double *
     PD_TRY(field_grad_inputs(f, level, &psi, &N, &K, &marginal, &mu, &sig, &wscale, &m_w));
     PD_REQUIRE(K <= kFgMaxK, "n_modes above %d", kFgMaxK);
     cudaStream_t s = (cudaStream_t)stream;
-    const int NT = fg_nodes(K), nchunks = (int)((N + NT - 1) / NT);
+    const int NT = fg_nodes(K), tiles = (int)((N + NT - 1) / NT), per = (tiles + kFgChunks - 1) / kFgChunks,
+              nchunks = (tiles + per - 1) / per;
     PD_REQUIRE(B <= 65535, "at most 65535 samples per call");
+    const size_t each = (size_t)nchunks * K * sizeof(double);  // partials of a sample
+    const int group = std::min<long long>(B, std::max<long long>(1, (long long)(kFgScratch / each / kFgSamples)) * kFgSamples);
     Scratch part;
-    PD_TRY(scratch_alloc(part, (size_t)B * nchunks * K * sizeof(double), s));
+    PD_TRY(scratch_alloc(part, group * each, s));
     PD_CHECK_CUDA(cudaFuncSetAttribute(k_field_grad_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)fg_smem(kFgMaxK, fg_nodes(kFgMaxK))));
-    k_field_grad_partial<<<dim3(nchunks, (B + kFgSamples - 1) / kFgSamples), kFgThreads, fg_smem(K, NT), s>>>(
-        N, K, B, NT, psi, xi, dJ_ds0, marginal, mu, sig, wscale, m_w, nchunks, (double *)part.p);
-    PD_CHECK_LAUNCH();
-    k_field_grad_sum<<<dim3((K + 31) / 32, B), 256, 0, s>>>(K, nchunks, (const double *)part.p, dJ_dxi);
-    PD_CHECK_LAUNCH();
+    for (int b = 0; b < B; b += group) {
+        const int n = std::min(group, B - b);
+        k_field_grad_partial<<<dim3(nchunks, (n + kFgSamples - 1) / kFgSamples), kFgThreads, fg_smem(K, NT), s>>>(
+            N, K, n, NT, per, psi, xi + (size_t)b * K, dJ_ds0 + (size_t)b * N, marginal, mu, sig, wscale, m_w, nchunks,
+            (double *)part.p);
+        PD_CHECK_LAUNCH();
+        k_field_grad_sum<<<dim3((K + 31) / 32, n), 256, 0, s>>>(K, nchunks, (const double *)part.p, dJ_dxi + (size_t)b * K);
+        PD_CHECK_LAUNCH();
+    }
     PD_CHECK_CUDA(cudaStreamSynchronize(s));
     return PD_OK;
 }
