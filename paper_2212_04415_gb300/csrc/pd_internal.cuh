@@ -65,8 +65,8 @@ struct Scratch {
     }
 };
 int scratch_alloc(Scratch &h, size_t bytes, cudaStream_t s);
-// A state or a field is made / destroyed: with the last one gone, the memory
-// that the current device's pool holds unused goes back to the device.
+// A state or a field is made / destroyed: with the last one gone, the memory that
+// the devices' pools hold unused goes back to them.
 void scratch_hold();
 void scratch_release();
 

@@ -2,8 +2,13 @@
 // memory pool per device, made at the first use: allocation and release are
 // ordered on the call's stream, so calls on several threads and streams never
 // share memory in use, and the pool keeps at most kKeep bytes unused (the
-// rest goes back to the device at the next synchronisation; all of it when the
-// last state or field is destroyed).
+// rest goes back to the device at the next synchronisation; all of it, on every
+// device, when the last state or field is destroyed). A pool goes with the
+// context that it was made in: after a cudaDeviceReset its handle is dropped,
+// never used, and the next call makes another (looking the context up: below 1
+// us a call).
+#include <cuda.h>
+
 #include <atomic>
 #include <mutex>
 
@@ -15,34 +20,87 @@ namespace {
 constexpr uint64_t kKeep = 64ull << 20;
 constexpr int kMaxDev = 64;
 std::mutex g_mu;
-cudaMemPool_t g_pool[kMaxDev] = {};
+struct Pool {
+    cudaMemPool_t pool = nullptr;
+    unsigned long long context = 0;
+} g_pool[kMaxDev];
 std::atomic<long> g_handles{0};  // live states and fields
 
-cudaMemPool_t pool_of(int dev, bool make) {
+struct Driver {
+    CUresult (*device)(CUdevice *, int) = nullptr;
+    CUresult (*state)(CUdevice, unsigned *, int *) = nullptr;
+    CUresult (*retain)(CUcontext *, CUdevice) = nullptr;
+    CUresult (*release)(CUdevice) = nullptr;
+    CUresult (*id)(CUcontext, unsigned long long *) = nullptr;
+    template <class F>
+    static bool get(const char *name, F &f) {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        f = (F)p;
+        return true;
+    }
+    bool ok;
+    Driver()
+        : ok(get("cuDeviceGet", device) && get("cuDevicePrimaryCtxGetState", state) &&
+             get("cuDevicePrimaryCtxRetain", retain) && get("cuDevicePrimaryCtxRelease", release) &&
+             get("cuCtxGetId", id)) {}
+};
+
+// Id of the device's primary context, unique in the life of the process; 0: it
+// is not active (the device was reset, not used yet, or is used through other
+// contexts only).
+unsigned long long context_of(int dev) {
+    static const Driver d;
+    CUdevice cd;
+    CUcontext c;
+    unsigned flags;
+    int active = 0;
+    unsigned long long id = 0;
+    if (!d.ok || d.device(&cd, dev) != CUDA_SUCCESS || d.state(cd, &flags, &active) != CUDA_SUCCESS || !active ||
+        d.retain(&c, cd) != CUDA_SUCCESS)
+        return 0;
+    if (d.id(c, &id) != CUDA_SUCCESS) id = 0;
+    d.release(cd);
+    return id;
+}
+
+// The device's pool, if the context that it was made in still stands (g_mu held).
+cudaMemPool_t live_pool(int dev) {
+    Pool &g = g_pool[dev];
+    if (g.pool && g.context != context_of(dev)) g = Pool{};
+    return g.pool;
+}
+
+cudaMemPool_t pool_of(int dev) {
     if (dev < 0 || dev >= kMaxDev) return nullptr;
     std::lock_guard<std::mutex> lock(g_mu);
-    if (!g_pool[dev] && make) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        uint64_t keep = kKeep;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
-        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaMemPoolDestroy(pool);
-            return nullptr;
-        }
-        g_pool[dev] = pool;
+    if (cudaMemPool_t p = live_pool(dev)) return p;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kKeep;
+    if (cudaFree(nullptr) != cudaSuccess || cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return nullptr;
     }
-    return g_pool[dev];
+    g_pool[dev].pool = pool;
+    g_pool[dev].context = context_of(dev);
+    return pool;
 }
 }  // namespace
 
 int scratch_alloc(Scratch &h, size_t bytes, cudaStream_t s) {
     int dev = 0;
     PD_CHECK_CUDA(cudaGetDevice(&dev));
-    cudaMemPool_t pool = pool_of(dev, true);
+    cudaMemPool_t pool = pool_of(dev);
     cudaError_t e = pool ? cudaMallocFromPoolAsync(&h.p, bytes ? bytes : 1, pool, s) : cudaErrorMemoryAllocation;
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -58,10 +116,9 @@ void scratch_hold() { ++g_handles; }
 
 void scratch_release() {
     if (--g_handles > 0) return;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return;
-    cudaMemPool_t pool = pool_of(dev, false);
-    if (pool) cudaMemPoolTrimTo(pool, 0);
+    std::lock_guard<std::mutex> lock(g_mu);
+    for (int dev = 0; dev < kMaxDev; ++dev)
+        if (g_pool[dev].pool && live_pool(dev)) cudaMemPoolTrimTo(g_pool[dev].pool, 0);
 }
 
 }  // namespace pdi
