@@ -5,8 +5,7 @@
 // rest goes back to the device at the next synchronisation; all of it, on every
 // device, when the last state or field is destroyed). A pool goes with the
 // context that it was made in: after a cudaDeviceReset its handle is dropped,
-// never used, and the next call makes another (looking the context up: below 1
-// us a call).
+// never used, and the next call makes another.
 #include <cuda.h>
 
 #include <atomic>
@@ -22,7 +21,8 @@ constexpr int kMaxDev = 64;
 std::mutex g_mu;
 struct Pool {
     cudaMemPool_t pool = nullptr;
-    unsigned long long context = 0;
+    CUcontext context = nullptr;  // the device's primary context, nullptr where it is not the one in use
+    unsigned long long id = 0;    // its id when the pool was made, unique in the life of the process
 } g_pool[kMaxDev];
 std::atomic<long> g_handles{0};  // live states and fields
 
@@ -51,28 +51,18 @@ struct Driver {
              get("cuCtxGetId", id)) {}
 };
 
-// Id of the device's primary context, unique in the life of the process; 0: it
-// is not active (the device was reset, not used yet, or is used through other
-// contexts only).
-unsigned long long context_of(int dev) {
+const Driver &driver() {
     static const Driver d;
-    CUdevice cd;
-    CUcontext c;
-    unsigned flags;
-    int active = 0;
-    unsigned long long id = 0;
-    if (!d.ok || d.device(&cd, dev) != CUDA_SUCCESS || d.state(cd, &flags, &active) != CUDA_SUCCESS || !active ||
-        d.retain(&c, cd) != CUDA_SUCCESS)
-        return 0;
-    if (d.id(c, &id) != CUDA_SUCCESS) id = 0;
-    d.release(cd);
-    return id;
+    return d;
 }
 
-// The device's pool, if the context that it was made in still stands (g_mu held).
+// The device's pool, if the context that it was made in still stands (g_mu
+// held). A device's primary context keeps its handle through a reset; its id
+// changes, or it has none.
 cudaMemPool_t live_pool(int dev) {
     Pool &g = g_pool[dev];
-    if (g.pool && g.context != context_of(dev)) g = Pool{};
+    unsigned long long id = 0;
+    if (g.pool && g.context && (driver().id(g.context, &id) != CUDA_SUCCESS || id != g.id)) g = Pool{};
     return g.pool;
 }
 
@@ -91,8 +81,17 @@ cudaMemPool_t pool_of(int dev) {
         cudaMemPoolDestroy(pool);
         return nullptr;
     }
-    g_pool[dev].pool = pool;
-    g_pool[dev].context = context_of(dev);
+    Pool &g = g_pool[dev];
+    g.pool = pool;
+    const Driver &d = driver();
+    CUdevice cd;
+    unsigned flags;
+    int active = 0;
+    if (d.ok && d.device(&cd, dev) == CUDA_SUCCESS && d.state(cd, &flags, &active) == CUDA_SUCCESS && active &&
+        d.retain(&g.context, cd) == CUDA_SUCCESS) {
+        if (d.id(g.context, &g.id) != CUDA_SUCCESS) g.context = nullptr;
+        d.release(cd);
+    }
     return pool;
 }
 }  // namespace
