@@ -46,11 +46,11 @@ L2_FLUSH_BYTES = 256 << 20
 # this program), reported only while the kernel's sources are the ones captured
 # (compared as code: comments and whitespace do not count).
 NCU_STEP_TRAFFIC = {
-    "bytes": 18_029_568 + 256,
+    "bytes": 18_029_568 + 0,
     "sources": {
         "paper_2212_04415_gb300/csrc/pd_stencil_kernel.cuh": "998973ad0ea7f1974c51d00bd84edc0392e881a46b0e3bbd44d18b3befad0683",
-        "paper_2212_04415_gb300/csrc/pd_stencil.cu": "ea63ff1137159bd91e0fd55b5876cd5c0f80bc669f835122e0daf2ba11316153",
-        "paper_2212_04415_gb300/csrc/pd_device.cuh": "d09ae61e086ec6d7013b8bc7d9e420eb5e98f49aadd79b83500e9fbe220d7324",
+        "paper_2212_04415_gb300/csrc/pd_stencil.cu": "83db71201f8e884366736fe6816216e25d4e6aa49d1328f74a1755166e43e419",
+        "paper_2212_04415_gb300/csrc/pd_device.cuh": "310760186eafa5222065f7a1ba776bbb47d521c2dd069c3a3542677813adcbd9",
     },
 }
 

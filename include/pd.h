@@ -299,7 +299,7 @@ PD_API int pd_run_to_peak(pd_state *st, int32_t max_steps, double *peak, int32_t
  * copies of the state's arrays (64 N + 520 N bytes with whole bricks), 16 k N
  * bytes of FP32 node records, 128 N bytes of adjoint state and masks, and per
  * bond whose damage grows in the run (only those carry a damage adjoint)
- * 4 (k + 1) + 12 bytes; for FP64-path states checkpoints of
+ * 4 (k + 1) + 12 bytes (16 where a sample has more than 2^32 damage words); for FP64-path states checkpoints of
  * (n_steps / k + 2) (6N + n_b) doubles, adjoint state 12 N doubles, the
  * segment's trajectory k 3N + (k + 1) n_b doubles and n_b doubles of damage
  * adjoint; for other mixed-path states those checkpoints and adjoint state,

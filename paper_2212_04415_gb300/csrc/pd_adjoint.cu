@@ -170,12 +170,11 @@ __global__ void __launch_bounds__(256) k_adj_bonds(const AdjArgs a, const double
     }
 }
 
-// FP32 variant for states of the mixed path (their trajectory is FP32-class
-// already): the same terms per bond in FP32 on FP32 copies of u^n and lamF^n;
-// per-lane partial sums in FP32 (a lane takes ~4 of a node's bonds), warp sums
-// and the carried damage adjoint in FP64. GB300 runs FP64 at a small fraction
-// of the FP32 rate, so this keeps the FP64 pipe to a few operations per bond.
-// (The derivatives of the law in FP32 are in pd_adjoint.cuh.)
+// Mixed-path states (their trajectory is FP32-class already): the same terms
+// per bond in FP32 on FP32 copies of u^n and lamF^n, which keeps them off the
+// FP64 pipe (k_adj_bonds_f32 below; the law's derivatives in FP32 are in
+// pd_adjoint.cuh). On the compile-time stencil with ascending rows they take
+// pd_adjoint_stencil.cu instead.
 
 // Node records of the mixed path at one step: (u, s0) with u = u_hi + u_lo
 // rounded to FP32, from the state's double-float gather records.

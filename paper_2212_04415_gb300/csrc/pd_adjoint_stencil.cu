@@ -291,8 +291,10 @@ struct AdjTab {
 };
 
 // Tiles of 8 x TY x TZ nodes (a warp takes 4 rows along y) and a halo of 3;
-// TY TZ <= 40, so that three blocks of at most 320 threads share an SM (64
-// registers a thread, at most 96 KB of records a block).
+// TY TZ <= 40, so that the registers of three blocks of at most 320 threads fit
+// an SM (64 a thread). Three blocks share it up to about 2,200 cells of records
+// (74 KB with the table), two up to the most, 3,072 (96 KB), which thin grids
+// reach.
 constexpr int kAdjThreads = 320;
 constexpr int kMaxCells = 3072;  // 96 KB of records
 struct AdjTile {

@@ -31,7 +31,9 @@
 //   224,000 x 100                      53    (66)
 //   28,000 x 1                         20    (23)
 //   28,000 x 256                       29    (31)
-// (286 MB of Psi and fields take 42 us at the copy rate.)
+// (286 MB of Psi and fields take 42 us at the copy rate. A call for 28,000 x 1, with
+// the drawing of its coefficients and the host's part, shows no gain: 30 to 38 us
+// against 32 to 36, runs of either differing by 7 to 14 %.)
 // Every wait on an mbarrier has an iteration limit; on expiry the CTA records
 // an error, writes NaN into its remaining tiles and still waits (bounded) for
 // its own copies and MMAs before it frees tensor memory.

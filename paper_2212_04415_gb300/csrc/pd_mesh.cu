@@ -6,7 +6,7 @@
 // list is a pure integer function of the grid (bit-exact, no atomics).
 //
 // Four launches (grid of 448,000 nodes, 50M bonds, GB300, count and fill calls
-// together with their two host synchronisations: 0.19 ms; with one thread
+// together with their three host synchronisations: 0.24 ms; with one thread
 // walking a node's candidate box for both passes and a one-block scan of every
 // row: 4.6 ms):
 //   k_row_counts  a thread per node counts whole x-ranges of the stencil's
