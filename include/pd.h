@@ -305,7 +305,8 @@ PD_API int pd_run_to_peak(pd_state *st, int32_t max_steps, double *peak, int32_t
  * adjoint; for other mixed-path states those checkpoints and adjoint state,
  * 16 k N + 4 (k + 1) S bytes of FP32 trajectory (S the slots of a sliced-ELL
  * copy of the rows, about n_b), 8 S bytes of double-float damage adjoint and S
- * bytes of damage history codes.
+ * bytes of damage history codes (states on the stencil path take these too
+ * where the copies do not fit: bricks that reach far past a thin grid).
  * Arithmetic: FP64 for FP64-path states; for mixed-path states the bond terms
  * in FP32 on the FP32 trajectory (the forward path's own precision class),
  * the damage adjoint in double-float, the node sums in FP64. The states come

@@ -626,8 +626,13 @@ extern "C" int pd_adjoint(pd_state *st, int32_t n_steps, int32_t ckpt_every, int
         a.L0q[q] = (float)L0;
         a.iL0q[q] = q ? (float)(1.0 / L0) : 0.f;
     }
-    if (st->mat.precision == PD_PREC_MIXED && st->stencil && st->st_sorted)
-        return adjoint_stencil(st, a, n_steps, k, steps.data(), grad_s0, grad_kappa, R_obs, stream);
+    if (st->mat.precision == PD_PREC_MIXED && st->stencil && st->st_sorted) {
+        const int rc = adjoint_stencil(st, a, n_steps, k, steps.data(), grad_s0, grad_kappa, R_obs, stream);
+        // Its checkpoints hold whole bricks: where the grid fills them badly they
+        // can be larger than in CSR order, which the general path takes (the
+        // state is as it was).
+        if (rc != PD_ERR_OOM) return rc;
+    }
 
     DevBuf<double> ck_u, ck_v, ck_d, tr_u, tr_d, lu, lun, lv, lF, ld, rbuf;
     // the mixed path's FP32 trajectory: node records (u, s0) per step, damage
