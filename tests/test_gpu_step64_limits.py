@@ -80,3 +80,25 @@ def test_compressed_bonds(built_lib, shrink):
     Fo, do, _ = core.Model(w, orow, ocol).force(u, np.zeros(len(ocol)))
     assert not do.any() and np.isfinite(Fo).all()
     assert np.abs(F - Fo).max() <= 1e-12 * np.abs(Fo).max()
+
+
+def test_bonds_of_undefined_damage_carry_no_force(built_lib):
+    """Damage that is not a number, of either sign, is not below 1: such a bond counts as broken, as in the oracle."""
+    pd = built_lib
+    w = W.tiny_beam()
+    g = w.grid
+    orow, ocol = core.neighbours(g)
+    rng = np.random.default_rng(6)
+    d = np.where(rng.random(len(ocol)) < 0.2, rng.random(len(ocol)), 0.0)
+    d[::5], d[1::7], d[2::9] = np.nan, -np.float64(np.nan), 1.0
+    assert np.signbit(d).any() and np.isnan(d[0]) and not np.signbit(d[0])
+    u, _ = W.random_state(g.n_nodes, 1, 9)
+    row, col = pd.build_neighbours(g)
+    st = pd.State(g, row, col, w.mat, w.bc, batch=1, precision=pd.PREC_FP64)
+    st.reset(torch.full((1, g.n_nodes), 1e-4, device="cuda"))
+    st.load(_dev(u), _dev(np.zeros_like(u)), _dev(d[None]), step=0)
+    F = st.force().cpu().numpy()[0]
+    st.close()
+    Fo, _, _ = core.Model(w, orow, ocol).force(u[0], d.copy())
+    assert np.isfinite(Fo).all() and np.abs(Fo).max() > 0
+    assert np.abs(F - Fo).max() <= 1e-10 * np.abs(Fo).max()  # (stretches of 1e-5: the oracle's (|y| - |xi|) / |xi| cancels)
